@@ -57,15 +57,16 @@ rqmc_status common_checks(int s, int64_t N, int64_t offset, int M, int seq, int 
 }
 
 void set_reduction(Plan &pl, int nout, int threads, int ppt) {
+    const UnitShape u = unit_shape(pl.N, (uint32_t)pl.M, threads, ppt);
     pl.threads = threads;
-    pl.ppt = ppt;
+    pl.ppt = u.ppt;
     pl.nout = nout;
     RedParams &r = pl.red;
     r.nout = nout;
-    r.ppt = ppt;
-    r.tile = (uint32_t)(threads * ppt);
-    r.tiles_per_m = (uint32_t)((pl.N + r.tile - 1) / r.tile);
-    r.units = r.tiles_per_m * (uint32_t)pl.M;
+    r.ppt = u.ppt;
+    r.tile = u.tile;
+    r.tiles_per_m = u.tiles_per_m;
+    r.units = u.units;
     r.N = (uint32_t)pl.N;
 }
 
@@ -471,7 +472,7 @@ extern "C" rqmc_status rqmc_plan_set_launch(rqmc_plan *plan, int threads, int pa
     }
     int t = threads > 0 ? threads : plan->threads;
     int p = paths_per_thread > 0 ? paths_per_thread : plan->ppt;
-    if (t % 32 != 0 || t < 32 || t > 256 || p < 1 || p > 64) {
+    if (t % 32 != 0 || t < 32 || t > 256 || p < 1 || paths_per_thread > 64) {
         set_error("threads must be a multiple of 32 in 32..256, paths_per_thread in 1..64");
         return RQMC_EINVAL;
     }

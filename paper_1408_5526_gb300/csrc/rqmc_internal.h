@@ -8,6 +8,7 @@
 
 #include "../../include/rqmc.h"
 #include "rqmc_common.cuh"
+#include "units.h"
 
 namespace rqmc {
 
