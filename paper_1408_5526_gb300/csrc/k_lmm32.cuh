@@ -23,11 +23,10 @@
 // Layout.  Forward n of a strip of nf sits in slot NF - nf + n - 1, so the alive slots of a
 // step are always the last ones and no step runs over unused slots; slot k is fixed at the end
 // of step k.  Steps go in sub-blocks of GR: the step code of a sub-block is compiled for its
-// first slot and is one straight line, GR slots of which the dead ones are masked (their
-// constants come from an entry with s = 0 and H = 2^40, whose drift term vanishes) and then
-// every later slot.  Straight-line code is what makes the kernel fast: the updates' long chains
-// (ex2, rcp) overlap only inside a basic block, and a version that jumped into a chain of 8-slot
-// blocks ran at half the rate with the same instructions.  GR trades masked slots against code
+// first slot and is one straight line, GR slots of which the dead ones are masked (their drift
+// terms vanish, see below) and then every later slot.  Straight-line code is what makes the kernel
+// fast: the updates' long chains (ex2, rcp) overlap only inside a basic block, and a version that
+// jumped into a chain of 8-slot blocks ran at half the rate with the same instructions.  GR trades masked slots against code
 // size (NF^2 / (2 GR) updates).
 //
 // Payoffs.  A step leaves (delta L, D) of its forward (for the batch (L, delta D), the same product) in the warp's buffer; after 8 steps each
@@ -46,34 +45,43 @@ struct Lmm32Scal {
     float l_scale, d_scale;   // payoff (l_scale delta L - Ks)^+ d_scale D
 };
 
-// Constants in shared memory: P >= 2, entry k = (s, s, H, H) of slot k; P = 1, entry q =
-// (s, s, H, H) of slots (2q, 2q + 1) and entry NF/2 + q the same with slot 2q dead; then one
-// entry for dead slots; then x0[NF] = log2(delta L(0)).  Slots below NF - nf are never alive.
-constexpr float kLmmDeadH = 1.099511627776e12f;   // 2^40
+// Constants in shared memory: P >= 2, entry k = (s, s, H, H) of slot k, then one for dead slots; P = 1,
+// entry q = (s, s, H, H) of slots (2q, 2q + 1); then x0[NF] = log2(delta L(0)).  Slots below NF - nf
+// are never alive.
+//
+// A dead slot's state is not read: forwards fall without bound (2^-90 from a tiny initial value or a
+// volatility of some hundred percent), and 1 + 2^-X of one that is fixed must not overflow the
+// product that an alive neighbour's reciprocal comes from.  Its update reads X = -40 (FLAT and P = 1, drift
+// term s 2^-40), or the entry s = 0, H = 2^40 with a state that was cleared when it was fixed (P >= 2
+// with constants from memory, where selecting the state instead of the address took 40 forwards,
+// N = 65536, M = 64 from 1.527 to 1.556 ms; as it is 1.535).
+constexpr float kLmmDeadX = -40.0f, kLmmDeadH = 1.099511627776e12f;   // 2^40
 template <int NF, int P>
 __host__ __device__ constexpr size_t lmm32_const_bytes() {
-    return (NF + 1) * sizeof(float4) + NF * sizeof(float);
+    return (P == 1 ? NF / 2 : NF + 1) * sizeof(float4) + NF * sizeof(float);
+}
+template <int NF, int P>
+__device__ __forceinline__ float *lmm32_x0(float4 *cst) {
+    return reinterpret_cast<float *>(cst + (P == 1 ? NF / 2 : NF + 1));
 }
 template <int NF, int P>
 __device__ __forceinline__ void lmm32_fill_constants(const LmmModel<float> &md, float4 *cst) {
-    float *x0 = reinterpret_cast<float *>(cst + NF + 1);
+    float *x0 = lmm32_x0<NF, P>(cst);
     const int sh = NF - md.nf;
     const float c = md.s_scale;
     for (int k = threadIdx.x; k < NF; k += blockDim.x) {
         const int n = k - sh;
-        const float s = n >= 0 ? md.sig[n] * c : 0.0f, H = lmm_fold_inv(s);
+        const float s = n >= 0 ? md.sig[n] * c : 0.0f, H = n >= 0 ? lmm_fold_inv(s) : 1.0f;
         x0[k] = n >= 0 ? md.X0[n] : 0.0f;
         if constexpr (P == 1) {
-            float *e = reinterpret_cast<float *>(cst + (k >> 1)) + (k & 1), *d = e + 2 * NF;
+            float *e = reinterpret_cast<float *>(cst + (k >> 1)) + (k & 1);
             e[0] = s;
             e[2] = H;
-            d[0] = (k & 1) ? s : 0.0f;
-            d[2] = (k & 1) ? H : kLmmDeadH;
         } else {
             cst[k] = make_float4(s, s, H, H);
         }
     }
-    if (threadIdx.x == 0) cst[NF] = make_float4(0.0f, 0.0f, kLmmDeadH, kLmmDeadH);
+    if (P > 1 && threadIdx.x == 0) cst[NF] = make_float4(0.0f, 0.0f, kLmmDeadH, kLmmDeadH);
 }
 // One entry, loaded at the point of use (volatile: the compiler must not keep a strip's
 // constants in registers).
@@ -112,7 +120,7 @@ __host__ __device__ constexpr int lmm32_row() {
 // l_scale is 1.
 template <int NF, int GR, int SEQ, int P, bool ZG, bool FLAT>
 __device__ __forceinline__ void lmm32_path(PathGen<SEQ> (&pg)[P], const bool (&active)[P], const Lmm32Scal &sc,
-                                           const float4 *cst, const float *Ks, float *zb, float *wbuf, float *wacc,
+                                           float4 *cst, const float *Ks, float *zb, float *wbuf, float *wacc,
                                            float *wcmp, const int lane, const float *zg, size_t zN, uint32_t zi0) {
     constexpr int S = P == 1 ? 1 : P / 2;   // packed path pairs
     constexpr int NY = P == 1 ? NF / 2 : NF;
@@ -121,10 +129,10 @@ __device__ __forceinline__ void lmm32_path(PathGen<SEQ> (&pg)[P], const bool (&a
     static_assert(NF % GR == 0 && (GR % 8 == 0 || 8 % GR == 0), "whole sub-blocks");
     const int nK = sc.nK, sh = NF - sc.nf;
     const unsigned ca = (unsigned)__cvta_generic_to_shared(cst);
-    const f32x2 mhalf = dup2(-0.5f), fs = dup2(sc.s), fH = dup2(sc.H), fdead = dup2(kLmmDeadH);
+    const f32x2 mhalf = dup2(-0.5f), fs = dup2(sc.s), fH = dup2(sc.H);
     f32x2 X[S][NY];
     {
-        const float *x0 = reinterpret_cast<const float *>(cst + NF + 1);
+        const float *x0 = lmm32_x0<NF, P>(cst);
 #pragma unroll
         for (int k = 0; k < NY; ++k)
 #pragma unroll
@@ -178,20 +186,15 @@ __device__ __forceinline__ void lmm32_path(PathGen<SEQ> (&pg)[P], const bool (&a
                     W[s] = FLAT ? fma2(z, dup2(sc.zscale), dup2(-0.5f * sc.s)) : mul2(z, dup2(sc.zscale));
                 }
             }
+            // the state that slot k's drift term comes from
+            auto state = [&](const float x, const int k, const bool masked) { return (FLAT || P == 1) && masked && slot > k ? kLmmDeadX : x; };
             // slots 2q, 2q + 1; masked: some of them may be dead
             auto pair = [&](const int q, const bool masked) {
                 if constexpr (P == 1) {
                     Lmm32C c{fs, fH};
-                    if constexpr (FLAT) {
-                        if (masked)
-                            c.H = pack2(slot > 2 * q ? kLmmDeadH : sc.H, slot > 2 * q + 1 ? kLmmDeadH : sc.H);
-                    } else {
-                        unsigned a = ca + 16 * q;
-                        if (masked) a = slot > 2 * q + 1 ? ca + 16 * NF : slot > 2 * q ? a + 8 * NF : a;
-                        c = lmm32_lds(a);
-                    }
+                    if constexpr (!FLAT) c = lmm32_lds(ca + 16 * q);
                     f32x2 &x = X[0][q];
-                    const f32x2 e = pack2(ex2_approx(-lo2(x)), ex2_approx(-hi2(x)));
+                    const f32x2 e = pack2(ex2_approx(-state(lo2(x), 2 * q, masked)), ex2_approx(-state(hi2(x), 2 * q + 1, masked)));
                     const f32x2 d = fma2(e, c.H, c.H);
                     const float r = rcp_approx(lo2(d) * hi2(d));
                     const float w0 = fmaf(r, hi2(d), w);
@@ -204,20 +207,15 @@ __device__ __forceinline__ void lmm32_path(PathGen<SEQ> (&pg)[P], const bool (&a
                     }
                 } else {
                     Lmm32C c0{fs, fH}, c1{fs, fH};
-                    if constexpr (FLAT) {
-                        if (masked) {
-                            c0.H = slot > 2 * q ? fdead : fH;
-                            c1.H = slot > 2 * q + 1 ? fdead : fH;
-                        }
-                    } else {
+                    if constexpr (!FLAT) {
                         c0 = lmm32_lds(masked && slot > 2 * q ? ca + 16 * NF : ca + 32 * q);
                         c1 = lmm32_lds(masked && slot > 2 * q + 1 ? ca + 16 * NF : ca + 32 * q + 16);
                     }
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
                         f32x2 &xa = X[s][(2 * q) % NY], &xb = X[s][(2 * q + 1) % NY];
-                        const f32x2 e0 = pack2(ex2_approx(-lo2(xa)), ex2_approx(-hi2(xa)));
-                        const f32x2 e1 = pack2(ex2_approx(-lo2(xb)), ex2_approx(-hi2(xb)));
+                        const f32x2 e0 = pack2(ex2_approx(-state(lo2(xa), 2 * q, masked)), ex2_approx(-state(hi2(xa), 2 * q, masked)));
+                        const f32x2 e1 = pack2(ex2_approx(-state(lo2(xb), 2 * q + 1, masked)), ex2_approx(-state(hi2(xb), 2 * q + 1, masked)));
                         const f32x2 d0 = fma2(e0, c0.H, c0.H), d1 = fma2(e1, c1.H, c1.H), m = mul2(d0, d1);
                         const f32x2 r = pack2(rcp_approx(lo2(m)), rcp_approx(hi2(m)));
                         W[s] = fma2(r, d1, W[s]);
@@ -228,10 +226,12 @@ __device__ __forceinline__ void lmm32_path(PathGen<SEQ> (&pg)[P], const bool (&a
                             if (slot == 2 * q) {
                                 Xf[2 * s] = lo2(xa);
                                 Xf[(2 * s + 1) % P] = hi2(xa);
+                                if constexpr (!FLAT) xa = 0ull;
                             }
                             if (slot == 2 * q + 1) {
                                 Xf[2 * s] = lo2(xb);
                                 Xf[(2 * s + 1) % P] = hi2(xb);
+                                if constexpr (!FLAT) xb = 0ull;
                             }
                         }
                     }
