@@ -511,7 +511,6 @@ extern "C" rqmc_status rqmc_plan_execute(rqmc_plan *plan, double *theta_dev, voi
         case kAdjoint:
             e = plan->znorm ? launch_points(*plan, RQMC_NORMAL, plan->znorm, st, normals_ld(plan->N)) : cudaSuccess;
             if (e == cudaSuccess) e = launch_adjoint(*plan, st);
-            rows_grid = (unsigned)plan->grid;   // one flush per run of units
             break;
         default: set_error("plan kind cannot be executed"); return RQMC_EUNSUPPORTED;
     }
@@ -710,7 +709,10 @@ static rqmc_status make_adjoint(const rqmc_lmm_params *p, const double *strikes_
     const int nout = 1 + 2 * nf + nf * n_strikes;
     pl->nf_bucket = nf <= 40 ? 40 : 80;
     pl->checkpoint = 1;
-    set_reduction(*pl, nout, kAdjointThreads, 2);   // one pass of two paths per thread
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    set_reduction(*pl, nout, kAdjointThreads, adjoint_ppt((uint64_t)N, M, sms));
     AdjModel *md = new AdjModel();
     std::memset(md, 0, sizeof(AdjModel));
     pl->adjm = md;

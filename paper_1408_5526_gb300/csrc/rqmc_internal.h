@@ -261,6 +261,13 @@ inline int caplet64_threads(int n_fwd, int scheme) {
 // CTA size of the adjoint kernel: 64 threads of two paths, so that five CTAs (640 paths) fit the shared
 // memory of an SM with the state columns of an 80-forward strip.
 constexpr int kAdjointThreads = 64;
+// Points per thread and unit of an adjoint plan: two (one pass) for the balance of plans of few units,
+// up to eight, which spares partial rows and flushes, while 24 units per resident CTA (six per SM) remain.
+inline int adjoint_ppt(uint64_t N, int M, int sms) {
+    int ppt = 8;
+    while (ppt > 2 && N * (uint64_t)M < 24ull * 6 * (uint64_t)sms * kAdjointThreads * (uint64_t)ppt) ppt /= 2;
+    return ppt;
+}
 int occupancy_blocks(const Plan &pl);
 
 // ---- the caller's initial curve as forwards (eq. BL for bond prices); p points into itself
