@@ -294,52 +294,58 @@ static rqmc_status make_product(int s, int64_t N, int64_t offset, int M, rqmc_se
     if (rs != RQMC_OK) return rs;
     set_reduction(*pl, 1, 128, 1);
     const size_t es = prec == RQMC_FP32 ? 4 : 8;
-    std::vector<unsigned char> model((prec == RQMC_FP32 ? 8 : 41) * (size_t)s);
-    // fixed point: a_j >= 0, so that a factor lies in (0, 2], and a product bound below 2^8
-    double bound = 1.0;
+    std::vector<unsigned char> model((prec == RQMC_FP32 ? 8 : 49) * (size_t)s);
+    // Fixed point where it rounds no path's product f by more than FP64 does: a factor adds at most one
+    // unit of 2^-(63 - fx_shift), 0.58 in the root mean square, to f, and a chain of FP64 products
+    // f 2^-53 sqrt(2) 0.29 or more, so that the smallest f, prod a_j / (1 + a_j), must not fall below
+    // 1.41 2^(fx_shift - 10).
+    double bound = 1.0, least = 1.0;
     bool fixed = prec == RQMC_FP64;
     for (int j = 0; j < s; ++j) {
-        fixed = fixed && a_host[j] >= 0.0 && a_host[j] < 1e6;
+        fixed = fixed && a_host[j] > 0.0 && a_host[j] < 1e6;
         bound *= (2.0 + a_host[j]) / (1.0 + a_host[j]);
+        least *= a_host[j] / (1.0 + a_host[j]);
     }
-    fixed = fixed && bound < 256.0;
+    int fx_shift = 0;
+    while (fx_shift < 10 && std::ldexp(1.0, fx_shift) < bound) ++fx_shift;   // f below 2^fx_shift
+    fixed = fixed && least >= std::ldexp(1.41, fx_shift - 10);
     const bool halton = seq == RQMC_HALTON_RS || seq == RQMC_RASRAP;
     const std::vector<uint32_t> base = halton ? first_primes(s) : std::vector<uint32_t>();
     for (int j = 0; j < s; ++j) {
         const double ia = 1.0 / (1.0 + a_host[j]);
         if (es == 4) {
-            const float v[2] = {(float)(2.0 + a_host[j]), (float)ia};
+            const float v[2] = {(float)a_host[j], (float)ia};
             std::memcpy(&model[j * 4], &v[0], 4);
             std::memcpy(&model[(s + j) * 4], &v[1], 4);
         } else {
             const double invD = halton ? 1.0 / (double)halton_denominator(base[j]) : 0x1p-32;
-            const double v[3] = {(2.0 - 2.0 * invD) + a_host[j], ia, -4.0 * invD};
-            for (int k = 0; k < 3; ++k) std::memcpy(&model[(k * (size_t)s + j) * 8], &v[k], 8);
+            const double v[4] = {a_host[j], ia, -4.0 * invD, 2.0 - 2.0 * invD};
+            for (int k = 0; k < 4; ++k) std::memcpy(&model[(k * (size_t)s + j) * 8], &v[k], 8);
             // fixed point: num <= (D - 1) / 2 shifted to the top of 64 bits; the high product with fc is
-            // 4 num / (D (1 + a)) in 2^-61
+            // 4 num / (D (1 + a)) in 2^-62
             const unsigned long long D = halton ? halton_denominator(base[j]) : 1ull << 32;
             const int sh = __builtin_clzll(D) + 1;
             const long double a1 = 1.0L + (long double)a_host[j];
             const long double fa = (1.0L + a1 - 2.0L / (long double)D) / a1, fc = 4.0L / ((long double)D * a1);
-            const unsigned long long w[2] = {fixed ? (unsigned long long)(ldexpl(fa, 61) + 0.5L) : 0ull,
-                                             fixed ? (unsigned long long)(ldexpl(fc, 125 - sh) + 0.5L) : 0ull};
-            for (int k = 0; k < 2; ++k) std::memcpy(&model[((3 + k) * (size_t)s + j) * 8], &w[k], 8);
-            model[40 * (size_t)s + j] = (unsigned char)sh;
+            const unsigned long long w[2] = {fixed ? (unsigned long long)(ldexpl(fa, 62) + 0.5L) : 0ull,
+                                             fixed ? (unsigned long long)(ldexpl(fc, 126 - sh) + 0.5L) : 0ull};
+            for (int k = 0; k < 2; ++k) std::memcpy(&model[((4 + k) * (size_t)s + j) * 8], &w[k], 8);
+            model[48 * (size_t)s + j] = (unsigned char)sh;
         }
     }
     size_t moff = 0;
     rs = finish_plan(pl, model, 16, partial_capacity(*pl, 1), st, standalone, &moff);
     if (rs != RQMC_OK) { destroy(pl, st); return rs; }
     unsigned char *d = static_cast<unsigned char *>(pl->d_buf) + moff;
-    if (es == 4) pl->prod32 = ProductModel<float>{s, (const float *)d, (const float *)(d + 4 * s), nullptr};
+    if (es == 4) pl->prod32 = ProductModel<float>{s, (const float *)d, (const float *)(d + 4 * s)};
     else {
-        pl->prod64 = ProductModel<double>{s, (const double *)d, (const double *)(d + 8 * s), (const double *)(d + 16 * s)};
+        pl->prod64 = ProductModel<double>{s, (const double *)d, (const double *)(d + 8 * s), (const double *)(d + 16 * s),
+                                          (const double *)(d + 24 * s)};
         if (fixed) {
-            pl->prod64.fx_shift = 0;
-            while (std::ldexp(1.0, pl->prod64.fx_shift) < bound) ++pl->prod64.fx_shift;   // product below 2^fx_shift
-            pl->prod64.fa = reinterpret_cast<const unsigned long long *>(d + 24 * (size_t)s);
-            pl->prod64.fc = reinterpret_cast<const unsigned long long *>(d + 32 * (size_t)s);
-            pl->prod64.fs = d + 40 * (size_t)s;
+            pl->prod64.fx_shift = fx_shift;
+            pl->prod64.fa = reinterpret_cast<const unsigned long long *>(d + 32 * (size_t)s);
+            pl->prod64.fc = reinterpret_cast<const unsigned long long *>(d + 40 * (size_t)s);
+            pl->prod64.fs = d + 48 * (size_t)s;
         }
     }
     pl->launches = 1;

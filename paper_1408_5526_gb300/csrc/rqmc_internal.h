@@ -60,18 +60,20 @@ struct MbsModel {
     const T *ck;             // [months + 1] remaining-annuity factors c_k (device)
 };
 
-// |4 x - 2| = 2 - 4 q from either side (q = min(x, 1 - x)), so a factor is (ca - 4 q) inv; in FP64 4 q is
-// taken from the integer numerator, ca + cn num.
+// |4 x - 2| = 2 - 4 q from either side (q = min(x, 1 - x)), so a factor is ((2 - 4 q) + a) inv, added in
+// this order (2 + a would round before a small 2 - 4 q + a is formed); in FP64 2 - 4 q is taken from the
+// integer numerator, c2 + cn num.
 template <typename T>
 struct ProductModel {
     int s;
-    const T *ca;             // [s] 2 + a_j, in FP64 less 4 (1/2) / D_j (device)
+    const T *a;              // [s] (device)
     const T *inv1pa;         // [s] 1/(1+a_j) (device)
-    const T *cn;             // [s] -4 / D_j (device; FP64)
-    // FP64 in 64-bit fixed point (fx_shift >= 0): factor fa - high(fc, num << fs) in 2^-61, running
+    const T *cn = nullptr;   // [s] -4 / D_j (device; FP64)
+    const T *c2 = nullptr;   // [s] 2 - 2 / D_j (device; FP64)
+    // FP64 in 64-bit fixed point (fx_shift >= 0): factor fa - high(fc, num << fs) in 2^-62, running
     // product in 2^-(63 - fx_shift)
     int fx_shift = -1;
-    const unsigned long long *fa = nullptr, *fc = nullptr;   // [s] (2 + a_j - 2/D_j)/(1 + a_j), 4 2^(64-fs)/(D_j (1 + a_j)), in 2^-61 (device)
+    const unsigned long long *fa = nullptr, *fc = nullptr;   // [s] (2 + a_j - 2/D_j)/(1 + a_j), 4 2^(64-fs)/(D_j (1 + a_j)), in 2^-62 (device)
     const unsigned char *fs = nullptr;                       // [s]
 };
 
