@@ -292,7 +292,10 @@ static rqmc_status make_product(int s, int64_t N, int64_t offset, int M, rqmc_se
     rqmc_plan *pl = nullptr;
     rqmc_status rs = new_plan(kProduct, s, N, offset, M, seq, seed, prec, &pl);
     if (rs != RQMC_OK) return rs;
-    set_reduction(*pl, 1, 128, 1);
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    set_reduction(*pl, 1, 128, product_ppt((uint64_t)N, M, sms));
     const size_t es = prec == RQMC_FP32 ? 4 : 8;
     std::vector<unsigned char> model((prec == RQMC_FP32 ? 8 : 49) * (size_t)s);
     // Fixed point where it rounds no path's product f by more than FP64 does: a factor adds at most one

@@ -254,6 +254,16 @@ inline int mbs_run_threads(uint64_t N, int M, int seq, int sms) {
     return t;
 }
 
+// Points per thread of product plans (128 threads): one while all points are in flight at once (2048 per
+// SM), which spreads the smallest plans evenly; then more, as every tile ends in a flush, a fence and
+// an atomic.  s = 8, us at one | two | four, FP64 random-start Halton: N M = 2^17 26.3 | 27.8 | 30.0, 2^19
+// 49.4 | 43.5 | 45.6, 2^22 253 | 238 | 237, 2^25 2003 | 1892 | 1837; FP32 Philox 20.0 | 20.1 | 20.2, 30.1 | 26.4 |
+// 26.3, 104 | 88 | 84, 687 | 571 | 509.
+inline int product_ppt(uint64_t N, int M, int sms) {
+    const uint64_t per_sm = N * (uint64_t)M / (uint64_t)sms;
+    return per_sm <= 2048 ? 1 : per_sm <= 8192 ? 2 : 4;
+}
+
 // CTA size of FP64 caplet plans: the fixed-point kernel keeps a path's forwards in shared memory
 // (k_lmm64.cuh), the floating-point kernel in registers.
 inline int caplet64_threads(int n_fwd, int scheme) {
