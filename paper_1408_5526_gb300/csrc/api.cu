@@ -417,7 +417,8 @@ static rqmc_status make_mbs(const rqmc_mbs_params *p, int64_t N, int64_t offset,
         int dev = 0, sms = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (const int t = mbs_run_threads((uint64_t)N, M, seq, sms)) set_reduction(*pl, 1, t, 8);
+        const int t = mbs_run_threads((uint64_t)N, M, seq, sms);
+        if (t && mbs_run_takes(*pl, t, 8)) set_reduction(*pl, 1, t, 8);
     }
     const int Mm = p->months;
     const double v = 1.0 / (1.0 + p->i0);

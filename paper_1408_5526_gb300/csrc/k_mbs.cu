@@ -83,11 +83,19 @@ static cudaError_t launch_mbs_t(const Plan &pl, const MbsModel<T> &md, cudaStrea
 // The run kernel serves FP32 plans whose launch shape gives every thread whole runs of 8 points,
 // with the per-replication tables in shared memory and, for Sobol', warps whose 256 points start
 // at a multiple of 256 (the lanes' index bits are then the point's bits 3..7).  Other plans
-// (FP64, thousands of months, odd Sobol' offsets, small plans: see mbs_run_threads) take mbs_kernel.
+// (FP64, thousands of months, odd Sobol' offsets, small plans: see mbs_run_threads) take mbs_kernel, and
+// its launch shape: in the run kernel's, FP32 plans of 360 months, Sobol', N = 1024, M = 2, offset 13 took
+// 596 us instead of 290, Rasrap, 1500 months, N = 65536, M = 8 8.18 ms instead of 3.89.
 template <int SEQ>
-static bool mbs_run_applies(const Plan &pl) {
-    return pl.prec == RQMC_FP32 && pl.ppt % 8 == 0 && pl.threads <= kMbsRunThreads && (SEQ != kSobolDS || pl.offset % 256 == 0) &&
-           mbs_run_smem<SEQ>(pl.s, pl.threads, pl.mbs32.months) <= 96 * 1024;
+static bool mbs_run_applies(const Plan &pl, int threads, int ppt) {   // s = months
+    return pl.prec == RQMC_FP32 && ppt % 8 == 0 && threads <= kMbsRunThreads && (SEQ != kSobolDS || pl.offset % 256 == 0) &&
+           mbs_run_smem<SEQ>(pl.s, threads, pl.s) <= 96 * 1024;
+}
+
+bool mbs_run_takes(const Plan &pl, int threads, int ppt) {
+#define RQMC_L(S) mbs_run_applies<S>(pl, threads, ppt)
+    return RQMC_SEQ_DISPATCH(pl.seq, RQMC_L);
+#undef RQMC_L
 }
 
 template <int SEQ>
@@ -111,7 +119,7 @@ static cudaError_t launch_mbs_run(const Plan &pl, cudaStream_t st, unsigned *row
 
 template <int SEQ>
 static cudaError_t launch_mbs_seq(const Plan &pl, cudaStream_t st, unsigned *rows_grid) {
-    if (mbs_run_applies<SEQ>(pl)) return launch_mbs_run<SEQ>(pl, st, rows_grid);
+    if (mbs_run_applies<SEQ>(pl, pl.threads, pl.ppt)) return launch_mbs_run<SEQ>(pl, st, rows_grid);
     return pl.prec == RQMC_FP32 ? launch_mbs_t<float, SEQ>(pl, pl.mbs32, st) : launch_mbs_t<double, SEQ>(pl, pl.mbs64, st);
 }
 

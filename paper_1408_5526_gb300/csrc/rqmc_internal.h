@@ -246,6 +246,7 @@ __host__ __device__ constexpr int mbs_paths32(int seq) { return seq == 2 || seq 
 // run kernel | two (Sobol' four) paths, us: Rasrap M N = 262144 451 | 510, 196608 435 | 402;
 // Sobol' 8192 223 | 270; Philox 524288 514 | 593, 262144 324 | 307.
 constexpr int kMbsRunThreads = 256;
+bool mbs_run_takes(const Plan &pl, int threads, int ppt);   // whether a plan of this shape runs in it
 inline int mbs_run_threads(uint64_t N, int M, int seq, int sms) {
     const uint64_t least = seq == 2 || seq == 4 ? 0 : seq == 3 ? 400000 : 200000;
     if (N * (uint64_t)M < least) return 0;
