@@ -208,7 +208,7 @@ cudaError_t launch_batch_class(const BatchLaunch &bl, cudaStream_t st) {
     unsigned grid = (unsigned)std::min<unsigned long long>(bl.n_items[KIND], (unsigned long long)occ * sms);
     if (bl.znorm[KIND]) grid = std::min<unsigned>(grid, bl.zctas[KIND]);   // one normals buffer per CTA
     kern<<<grid, bl.threads, smem, st>>>(bl.insts, bl.items[KIND], bl.n_items[KIND], bl.counter + KIND, bl.partials,
-                                         bl.ppt, bl.stats, bl.stats_cap, bl.znorm[KIND], bl.zstride[KIND]);
+                                         bl.class_ppt[KIND], bl.stats, bl.stats_cap, bl.znorm[KIND], bl.zstride[KIND]);
     return cudaGetLastError();
 }
 

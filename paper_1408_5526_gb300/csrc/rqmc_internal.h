@@ -143,6 +143,7 @@ struct BatchLaunch {
     unsigned long long *stats;    // [kBatchClasses][stats_cap] CTA records: SM id, start, end (ns)
     uint32_t stats_cap;
     int threads, ppt;
+    int class_ppt[kBatchClasses];   // paths per thread of each class's items
     size_t smem[kBatchClasses];
     // per-CTA normals buffers of the strip classes (0 and 2): zctas CTAs of zstride floats
     // (the largest bucket of the class x the tile); the class's grid never exceeds zctas
