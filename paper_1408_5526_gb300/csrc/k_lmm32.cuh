@@ -314,29 +314,29 @@ __device__ __forceinline__ void lmm32_path(PathGen<SEQ> (&pg)[P], const bool (&a
             const float nKv = on ? -Ks[rw - k * nK] : 0.0f;
             const f32x2 nk2 = dup2(nKv);
             const float *src = wbuf + (k0 + k) * ROW;
-            f32x2 t0 = dup2(0.0f), t1 = dup2(0.0f);
-            if constexpr (P == 1) {   // two paths (delta L, D, delta L, D) per 16-byte load
-#pragma unroll 4
-                for (int l = part; l < 16; l += lpr) {
-                    const float4 a = reinterpret_cast<const float4 *>(src)[l];
-                    const f32x2 x = add2(pack2(a.x, a.z), nk2);
-                    t0 = fma2(pack2(fmaxf(lo2(x), 0.0f), fmaxf(hi2(x), 0.0f)), pack2(a.y, a.w), t0);
-                }
-            } else {
-#pragma unroll 4
-                for (int l = part; l < 32; l += lpr) {
+            // four accumulators of two halves, so that a chain is at most 8 additions
+            f32x2 tk[4] = {dup2(0.0f), dup2(0.0f), dup2(0.0f), dup2(0.0f)};
+            constexpr int NL = P == 1 ? 16 : 32;   // loads a row
 #pragma unroll
-                    for (int h = 0; h < P / 2; ++h) {
-                        const ulonglong2 q = reinterpret_cast<const ulonglong2 *>(src + 2 * P * l)[h];
-                        const f32x2 x = add2(q.x, nk2);
-                        const f32x2 pos = pack2(fmaxf(lo2(x), 0.0f), fmaxf(hi2(x), 0.0f));
-                        if (h & 1) t1 = fma2(pos, q.y, t1);
-                        else t0 = fma2(pos, q.y, t0);
+            for (int l = part; l < NL; l += 4 * lpr) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (P == 1) {   // two paths (delta L, D, delta L, D) per 16-byte load
+                        const float4 a = reinterpret_cast<const float4 *>(src)[l + k * lpr];
+                        const f32x2 x = add2(pack2(a.x, a.z), nk2);
+                        tk[k] = fma2(pack2(fmaxf(lo2(x), 0.0f), fmaxf(hi2(x), 0.0f)), pack2(a.y, a.w), tk[k]);
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < P / 2; ++h) {
+                            const ulonglong2 q = reinterpret_cast<const ulonglong2 *>(src + 2 * P * (l + k * lpr))[h];
+                            const f32x2 x = add2(q.x, nk2);
+                            tk[k] = fma2(pack2(fmaxf(lo2(x), 0.0f), fmaxf(hi2(x), 0.0f)), q.y, tk[k]);
+                        }
                     }
                 }
             }
-            t0 = add2(t0, t1);
-            float t = lo2(t0) + hi2(t0);
+            const f32x2 ta = add2(tk[0], tk[1]), tb = add2(tk[2], tk[3]);
+            float t = (lo2(ta) + lo2(tb)) + (hi2(ta) + hi2(tb));
             if (lpr > 1) t += __shfl_xor_sync(0xffffffffu, t, 1);
             if (lpr > 2) t += __shfl_xor_sync(0xffffffffu, t, 2);
             if (on && part == 0) {
