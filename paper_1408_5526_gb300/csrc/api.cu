@@ -40,6 +40,30 @@ static void keep_pool_cached(int dev) {
     });
 }
 
+// The pool of the adjoint's scratch (up to 250 MB a plan), one per device: up to 256 MiB stay with the
+// process between plans, so that a calibration step's two plans need no mapping, the rest goes back at the
+// next synchronisation.  Null where no pool can be made (then the device's default pool serves).
+static cudaMemPool_t adjoint_pool(int dev) {
+    static std::once_flag flags[64];
+    static cudaMemPool_t pools[64];
+    if (dev < 0 || dev >= 64) return nullptr;
+    std::call_once(flags[dev], [dev]() {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        uint64_t keep = 256ull << 20;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        pools[dev] = pool;
+    });
+    return pools[dev];
+}
+
 // ------------------------------------------------------------------ plan construction
 struct ModelHost {
     std::vector<unsigned char> bytes;   // model tables to copy after the generator tables
@@ -787,7 +811,8 @@ static rqmc_status make_adjoint(const rqmc_lmm_params *p, const double *strikes_
     pl->adjs.T = T;
     const size_t bytes = sizeof(float) * (rec_floats + xb_floats + rows) * T;
     void *buf = nullptr;
-    cudaError_t e = cudaMallocAsync(&buf, bytes, st);
+    cudaMemPool_t pool = adjoint_pool(pl->device);
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(&buf, bytes, pool, st) : cudaMallocAsync(&buf, bytes, st);
     if (e != cudaSuccess) { destroy(pl, st); set_error("adjoint: scratch allocation failed"); return RQMC_ENOMEM; }
     pl->adj_buf = buf;
     pl->adjs.store = static_cast<float *>(buf);
