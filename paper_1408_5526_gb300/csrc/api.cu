@@ -106,6 +106,17 @@ static bool caplets_draw_inside(int n_fwd, int seq, size_t zbytes) {
 // normals itself.
 static constexpr size_t kMaxNormalsBytes = 8ull << 30;
 
+// The buffer of a plan's normals.  Without memory for it the plan has none (znorm null), and its path kernel
+// draws the normals itself, as above the cap.
+static cudaError_t alloc_normals(Plan *pl, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = cudaMallocAsync(&pl->znorm, bytes, st);
+    if (e == cudaSuccess) return e;
+    pl->znorm = nullptr;
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return cudaSuccess;
+}
+
 // Allocates one device block: generator tables, model tables, status words, partials
 // (sized for the smallest tile, 32 paths, so launch knobs can change later).
 static rqmc_status finish_plan(Plan *pl, const std::vector<unsigned char> &model, size_t model_align,
@@ -410,14 +421,13 @@ static rqmc_status make_caplets(const rqmc_lmm_params *p, const double *strikes_
     // work of consecutive points, and the caplet kernel reads one per path and step
     const size_t zbytes = sizeof(float) * (size_t)M * (size_t)pl->s * normals_ld(pl->N);
     if (prec == RQMC_FP32 && zbytes <= kMaxNormalsBytes && !caplets_draw_inside(p->n_fwd, seq, zbytes)) {
-        cudaError_t e = cudaMallocAsync(&pl->znorm, zbytes, st);
+        cudaError_t e = alloc_normals(pl, zbytes, st);
         if (e == cudaSuccess && standalone) e = cudaStreamSynchronize(st);   // usable on every stream
         if (e != cudaSuccess) {
             destroy(pl, st);
-            set_error(std::string("device allocation failed (normals): ") + cudaGetErrorString(e));
-            return RQMC_ENOMEM;
+            return cuda_fail(e, "normals buffer");
         }
-        pl->launches = 3;
+        if (pl->znorm) pl->launches = 3;
     }
     *plan = pl;
     return RQMC_OK;
@@ -793,12 +803,10 @@ static rqmc_status make_adjoint(const rqmc_lmm_params *p, const double *strikes_
     // N = 2^18, M = 32).
     const size_t zbytes = sizeof(float) * (size_t)M * (size_t)pl->s * normals_ld(pl->N);
     if (pl->seq != kPhilox && zbytes <= kMaxNormalsBytes) {
-        cudaError_t ez = cudaMallocAsync(&pl->znorm, zbytes, st);
+        const cudaError_t ez = alloc_normals(pl, zbytes, st);
         if (ez != cudaSuccess) {
-            pl->znorm = nullptr;
             destroy(pl, st);
-            set_error(std::string("device allocation failed (normals): ") + cudaGetErrorString(ez));
-            return RQMC_ENOMEM;
+            return cuda_fail(ez, "normals buffer");
         }
     }
     pl->grid = adjoint_grid(*pl);
