@@ -250,7 +250,9 @@ int64_t rqmc_plan_output_size(const rqmc_plan *plan);
 rqmc_status rqmc_plan_batch_stats(rqmc_plan *plan, double *out_host, int n);
 /* Kernel launches one execute performs (for launch accounting). */
 int rqmc_plan_launches(const rqmc_plan *plan);
-/* Tuning knobs of a plan: threads per block and paths per thread (0 = keep). */
+/* Tuning knobs of a plan: threads per block and paths per thread (0 = keep).  Plans of more than 2^32
+ * units of threads x paths take more paths per thread.  FP64 log-Euler caplet plans of more than 128
+ * threads run in FP64 operations throughout, several times slower than the default's fixed point. */
 rqmc_status rqmc_plan_set_launch(rqmc_plan *plan, int threads, int paths_per_thread);
 /* The plan's launch shape (not in the paper): threads per block and paths per thread, for a
  * batch plan the tile its autotuner chose or read from its cache.  Host-only, no GPU work;

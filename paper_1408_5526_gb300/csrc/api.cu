@@ -499,7 +499,10 @@ extern "C" int64_t rqmc_plan_output_size(const rqmc_plan *plan) {
     return (int64_t)plan->M * plan->nout;
 }
 
-extern "C" int rqmc_plan_launches(const rqmc_plan *plan) { return plan ? plan->launches : 0; }
+extern "C" int rqmc_plan_launches(const rqmc_plan *plan) {
+    if (!plan) return 0;
+    return plan->launches + (plan->kind == kCaplets && caplets_fixed_point(*plan) ? 1 : 0);
+}
 
 extern "C" rqmc_status rqmc_plan_get_launch(const rqmc_plan *plan, int *threads, int *paths_per_thread) {
     if (!plan || !threads || !paths_per_thread) { set_error("plan and both outputs are required"); return RQMC_EINVAL; }

@@ -184,17 +184,23 @@ inline bool fx_fits(const LmmModel<double> &md, LmmFx &fx) {
     return sum < 100.0;
 }
 
+// Whether a plan's launch shape and paths let the fixed-point kernel run (smem: its shared memory).
+inline bool lmm64_applies(const Plan &pl, LmmFx &fx, size_t &smem) {
+    size_t a, b, c, d;
+    smem = lmm64_smem_layout(pl.gen, pl.threads, pl.lmm64.nf, pl.lmm64.nK, &a, &b, &c, &d);
+    return pl.prec == RQMC_FP64 && pl.scheme != RQMC_EULER && pl.threads <= 128 && pl.red.guard && smem <= 227 * 1024 &&
+           fx_fits(pl.lmm64, fx);
+}
+
 // Launches the fixed-point kernel where it applies (*launched); the caller launches the guarded
 // floating-point kernel behind it.
 template <int SEQ>
 static cudaError_t launch_lmm64(const Plan &pl, cudaStream_t st, bool *launched) {
     *launched = false;
     LmmFx fx;
-    if (pl.scheme == RQMC_EULER || pl.threads > 128 || !pl.red.guard || !fx_fits(pl.lmm64, fx)) return cudaSuccess;
+    size_t smem;
+    if (!lmm64_applies(pl, fx, smem)) return cudaSuccess;
     auto kern = lmm_caplet64_kernel<SEQ>;
-    size_t a, b, c, d;
-    const size_t smem = lmm64_smem_layout(pl.gen, pl.threads, pl.lmm64.nf, pl.lmm64.nK, &a, &b, &c, &d);
-    if (smem > 227 * 1024) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int occ = 0, dev = 0, sms = 0;

@@ -226,6 +226,8 @@ __host__ __device__ inline size_t normals_ld(uint64_t N) { return (size_t)((N + 
 cudaError_t launch_product(const Plan &pl, double *theta_dev, cudaStream_t st);
 // *rows_grid: 0, or the kernel's grid where it flushed once per run of units (see theta_kernel)
 cudaError_t launch_caplets(const Plan &pl, cudaStream_t st, unsigned *rows_grid);
+// a caplet plan's execute launches the FP64 fixed-point kernel (and the floating-point one behind it)
+bool caplets_fixed_point(const Plan &pl);
 cudaError_t launch_mbs(const Plan &pl, cudaStream_t st, unsigned *rows_grid);
 cudaError_t launch_theta(const Plan &pl, double *theta_dev, cudaStream_t st, unsigned rows_grid = 0);
 cudaError_t launch_adjoint(const Plan &pl, cudaStream_t st);
