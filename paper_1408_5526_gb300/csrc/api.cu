@@ -94,12 +94,17 @@ void set_reduction(Plan &pl, int nout, int threads, int ppt) {
     r.N = (uint32_t)pl.N;
 }
 
-// Small FP32 caplet plans draw their normals in the caplet kernel: one launch and one allocation less.
-// Measured, us per execute, inside | written beforehand: 10 forwards, N = 4096, M = 8 (1.3 MB) Sobol' 18 | 21,
-// Rasrap 19 | 33; M = 100 (16 MB) 36 | 38, 44 | 52; 20 forwards, M = 100 (33 MB) 74 | 70, 87 | 88; 40 forwards,
-// M = 8 (5 MB) Sobol' 46 | 44, Rasrap 52 | 54; 100 forwards, M = 8 192 | 157, 219 | 171.
+// Small FP32 caplet plans draw their normals in the caplet kernel: one launch and one allocation less.  Beyond
+// the lines below the point stream's shared digit and bit work wins, soonest for Sobol'; a path of more
+// than about 20 forwards leaves the kernel too few registers to draw in.  Measured, us per execute, inside |
+// written beforehand (forwards, MB of normals):
+//             10, 1.3      10, 5.2      10, 16       10, 66       20, 2.6      20, 8.2      20, 16       24, 16       40, 5.2
+//   Philox    19.5 | 22.0  19.0 | 26.2  35.2 | 39.4  103 | 106    26.2 | 27.0  30.2 | 36.1  51.8 | 51.6  64.3 | 61.9  47.6 | 43.5
+//   Rasrap    17.9 | 22.6  20.9 | 27.0  43.5 | 46.0  134 | 137    27.0 | 27.1  35.4 | 36.2  62.6 | 56.0  78.3 | 67.0  51.6 | 45.4
+//   Sobol'    16.9 | 19.6  20.6 | 22.4  37.3 | 35.2  113 | 93     25.0 | 24.9  33.1 | 31.1  55.7 | 47.5  68.3 | 58.9  47.5 | 41.4
 static bool caplets_draw_inside(int n_fwd, int seq, size_t zbytes) {
-    return zbytes <= (16u << 20) && n_fwd <= (seq == RQMC_SOBOL_DS || seq == RQMC_SOBOL_LMS ? 24 : 40);
+    const size_t most = seq == RQMC_PHILOX ? 32u << 20 : seq == RQMC_SOBOL_DS || seq == RQMC_SOBOL_LMS ? 6u << 20 : 12u << 20;
+    return n_fwd <= 20 && zbytes <= most;
 }
 
 // Largest normals buffer of an FP32 caplet plan; above it the caplet kernel generates its
