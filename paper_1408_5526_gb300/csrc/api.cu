@@ -65,11 +65,6 @@ static cudaMemPool_t adjoint_pool(int dev) {
 }
 
 // ------------------------------------------------------------------ plan construction
-struct ModelHost {
-    std::vector<unsigned char> bytes;   // model tables to copy after the generator tables
-    size_t off = 0;
-};
-
 rqmc_status common_checks(int s, int64_t N, int64_t offset, int M, int seq, int prec) {
     if (s < 1 || s > kMaxDims) { set_error("s must be in 1..4096"); return RQMC_EINVAL; }
     if (N < 1 || N > (int64_t(1) << 31)) { set_error("N must be in 1..2^31"); return RQMC_EINVAL; }

@@ -503,8 +503,6 @@ void batch_destroy(Plan &pl) {
     pl.batch = nullptr;
 }
 
-int batch_ppt(const Plan &pl) { return pl.batch ? pl.batch->bl.ppt : 0; }
-
 }  // namespace rqmc
 
 using namespace rqmc;

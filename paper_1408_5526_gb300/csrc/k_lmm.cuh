@@ -106,7 +106,7 @@ __device__ __forceinline__ T row_sum32(const T *row) {
 template <typename T>
 struct LmmScal {
     int nf, nK;
-    T dl, inv_dl, disc0, hc, sqhc;
+    T disc0, hc, sqhc;
 };
 
 // Fill the constants [NF] of (sigma_n, h sigma_n, cc_n, 0) and the initial state X0 (all threads of
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(256, lmm_min_blocks<NF, T>()) lmm_caplet_kerne
     lmm_fill_constants<NF, T>(md, cst, X0);
     if (threadIdx.x < kMaxStrikes) Ks[threadIdx.x] = md.dl * md.K[threadIdx.x];   // delta K
     zero_acc(acc, cmp, nw * nout);
-    const LmmScal<T> sc{md.nf, md.nK, md.dl, md.inv_dl, md.disc0, md.hc, md.sqhc};
+    const LmmScal<T> sc{md.nf, md.nK, md.disc0, md.hc, md.sqhc};
     uint32_t u0, u1;
     unit_range(r, u0, u1);
     GenView gv;
@@ -412,8 +412,7 @@ static cudaError_t launch_lmm_t(const Plan &pl, const LmmModel<T> &md, cudaStrea
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (occ < 1) occ = 1;
-    unsigned grid = (unsigned)std::min<unsigned long long>(pl.red.units, (unsigned long long)occ * sms);
-    if (pl.grid > 0) grid = (unsigned)std::min<unsigned long long>(pl.red.units, (unsigned long long)pl.grid);
+    const unsigned grid = (unsigned)std::min<unsigned long long>(pl.red.units, (unsigned long long)occ * sms);
     RedParams red = pl.red;
     if (!guarded) red.guard = nullptr;
     kern<<<grid, threads, smem, st>>>(g, md, red, ZG ? reinterpret_cast<const T *>(pl.znorm) : nullptr);

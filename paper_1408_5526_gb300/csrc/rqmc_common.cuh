@@ -378,10 +378,10 @@ __device__ __forceinline__ unsigned long long lower_num(PathGen<SEQ> &pg, int j)
                                                  : F(kRasrap))
 
 // ------------------------------------------------------------------ inverse normal CDF
-// erfinv(y)/y as a polynomial in w = -ln(4q(1-q)) (three branches, coefficients
-// fitted by fit_ndtri.py); Phi^-1(u) = -/+ sqrt(2) y P(w), y = 1 - 2q.  The FP32 routines
-// take the central branch as one polynomial in v = log2(q(1-q)) = -w/ln 2 - 2 that includes
-// the factor sqrt(2) (RQMC_NDTRI_V), so no scaling or shift is spent before or after it.
+// FP32: erfinv(y)/y as a polynomial in w = -ln(4q(1-q)) (three branches, coefficients
+// fitted by fit_ndtri.py); Phi^-1(u) = -/+ sqrt(2) y P(w), y = 1 - 2q.  The central branch
+// is one polynomial in v = log2(q(1-q)) = -w/ln 2 - 2 that includes the factor sqrt(2)
+// (RQMC_NDTRI_V), so no scaling or shift is spent before or after it.
 template <typename T, int N>
 __device__ __forceinline__ T horner(const T (&c)[N], T x) {
     T p = c[N - 1];
@@ -390,7 +390,7 @@ __device__ __forceinline__ T horner(const T (&c)[N], T x) {
     return p;
 }
 
-// sqrt(2) erfinv(y)/y from v = log2(q(1-q)): central polynomial for v > V_SPLIT (w < W_SPLIT),
+// sqrt(2) erfinv(y)/y from v = log2(q(1-q)): central polynomial for v > V_SPLIT (w < 5),
 // else the tail polynomials in sqrt(w).
 __device__ __forceinline__ float erfinv_central32(float v) {
     constexpr float V[] = RQMC_NDTRI_V;

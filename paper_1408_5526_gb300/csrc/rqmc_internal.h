@@ -235,7 +235,6 @@ cudaError_t launch_batch(const BatchLaunch &bl, int seq, cudaStream_t st);
 rqmc_status batch_execute(Plan &pl, double *theta_dev, cudaStream_t st);
 int64_t batch_output_size(const Plan &pl);
 void batch_destroy(Plan &pl);
-int batch_ppt(const Plan &pl);
 int adjoint_grid(const Plan &pl);
 // Paths per thread in lockstep in the FP32 MBS kernels (the MBS plans' paths per thread per
 // unit): four for Sobol' (the three extra points cost a few XORs of direction numbers each),
@@ -284,7 +283,6 @@ inline int adjoint_ppt(uint64_t N, int M, int sms) {
     while (ppt > 2 && N * (uint64_t)M < 24ull * 6 * (uint64_t)sms * kAdjointThreads * (uint64_t)ppt) ppt /= 2;
     return ppt;
 }
-int occupancy_blocks(const Plan &pl);
 
 // ---- the caller's initial curve as forwards (eq. BL for bond prices); p points into itself
 struct LmmCurve {
