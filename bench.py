@@ -60,14 +60,14 @@ def _peaks():
 
 
 def lmm_algorithmic_ops(nf, nK, paths):
-    """Source-level operations of one caplet plan execute (normals, paths, payoffs).
-    MUFU: ex2 + rcp per forward update; per step lg2 (inverse CDF) and ex2 + rcp
-    (fixed forward and numeraire).  Returned as SFU issue slots: on GB300 ex2 issues at
+    """Operations of one caplet plan execute (normals, paths, payoffs).
+    MUFU: ex2 and half an rcp (two forwards share one) per forward update; per step lg2
+    (inverse CDF) and ex2 + rcp (fixed forward and numeraire).  Returned as SFU issue slots: on GB300 ex2 issues at
     32 per SM per clock and rcp/lg2 at 16, so an ex2 counts half a slot.
     FP32 pipe: 4 per forward update (1 + e, drift, state), 16 per inverse CDF, 4 per step,
     4 per strike."""
     upd = nf * (nf + 1) // 2
-    n_ex2, n_rcp, n_lg2 = upd + nf, upd + nf, nf
+    n_ex2, n_rcp, n_lg2 = upd + nf, 0.5 * upd + nf, nf
     slots = 0.5 * n_ex2 + n_rcp + n_lg2
     fma = 4 * upd + nf * (16 + 4 + 4 * nK)
     return slots * paths, fma * paths
@@ -88,14 +88,14 @@ def mbs_algorithmic_ops(months, paths):
 
 def adjoint_algorithmic_ops(nf, d, paths):
     """Pathwise adjoint of a d-factor strip, per path: the forward sweep's nf(nf+1)/2 forward
-    updates (ex2 + rcp, 2 + 3d FP32), the reverse sweep's as many steps back (the pre-step state
-    reconstructed from the post-step one, 2 + d FP32, and its drift factor again, ex2 + rcp)
-    with their adjoint updates (3 + 7d FP32), the fixings' ex2 + rcp in both sweeps, and 2 nf d
-    inverse CDFs (the normals drawn in the forward sweep and regenerated in the reverse one,
-    lg2 + 17 FP32 each).  SFU slots and FP32 operations."""
+    updates (ex2 and half an rcp, which two slots share, 2 + 3d FP32), the reverse sweep's as many
+    steps back (the pre-step state reconstructed from the post-step one, 2 + d FP32, and its drift
+    factor again, ex2 + rcp) with their adjoint updates (3 + 7d FP32), the fixings' ex2 + rcp in
+    both sweeps, and nf d inverse CDFs (lg2 + 17 FP32 each; the reverse sweep needs no normals).
+    SFU slots and FP32 operations."""
     upd = nf * (nf + 1) // 2
-    slots = 1.5 * (2 * upd + 2 * nf) + 2 * nf * d
-    fma = (2 + 3 * d) * upd + (2 + d) * upd + (3 + 7 * d) * upd + 2 * nf * d * 17
+    slots = (1.0 + 1.5) * upd + 1.5 * 2 * nf + nf * d
+    fma = (2 + 3 * d) * upd + (2 + d) * upd + (3 + 7 * d) * upd + nf * d * 17
     return slots * paths, fma * paths
 
 

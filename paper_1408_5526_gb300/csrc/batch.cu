@@ -314,7 +314,7 @@ static int autotune(BatchPlan &bp) {
     if (it != kv.end() && it->second >= 1 && it->second <= 16) return it->second;
     int best = 4;
     float best_ms = 1e30f;
-    for (int ppt : {4, 8, 16}) {   // multiples of every bucket's paths per thread in lockstep
+    for (int ppt : {4, 8, 16}) {   // multiples of every strip bucket's paths per thread in lockstep
         if (setup_launch(bp, 256, ppt, true) != RQMC_OK) continue;
         const float ms = time_launch(bp);
         kv[key + "|us_ppt" + std::to_string(ppt)] = (int)std::lround(1000.0 * ms);   // the candidate's time

@@ -3,7 +3,7 @@
 // The FP64 pipe of this GPU starts two operations per SM and clock, so one FP64 forward update
 // (exp, division, four more) takes it about 14 clocks per path.  The 32-bit integer pipes take a
 // 64-bit high product in an eighth of a clock.  The log-forward X = log2(delta L) is therefore
-// held as a signed integer in units of 2^-55 (eight times finer than a double near X = -6), and
+// held as a signed integer in units of 2^-55 (32 times finer than a double near X = -6), and
 //   t = 2^-|X|  by a table of 2^(-i/2048) and a degree-4 polynomial (Tang's method),
 //   rho = 1 / (1 + t)  from the FP32 reciprocal by one second-order Newton step on integers,
 // each exact to about 2^-56, give delta L / (1 + delta L) = rho (X >= 0) or 1 - rho.

@@ -389,7 +389,7 @@ __host__ __device__ __forceinline__ size_t lmm32_smem_layout(const GenParams &g,
 }
 
 // The caplet kernel of FP32 log-Euler plans.  A CTA's warps keep their accumulators over the
-// CTA's consecutive units of one replication and write one row at the last of them (flush_run).
+// CTA's consecutive units of one replication and write one row at the last of them (run_ends).
 template <int NF, int SEQ, bool ZG, bool FLAT>
 __global__ void __launch_bounds__(256, lmm32_min_blocks<NF>())
     lmm_caplet32_kernel(const GenParams g, const LmmModel<float> md, const RedParams r, const float *__restrict__ zg) {

@@ -7,7 +7,10 @@
 // within one unit.  Within a unit each warp accumulates its per-step payload in shared
 // memory; at the end of the unit the warps' accumulators are added in double in warp
 // order and written to partials[u][o].  No float atomics: the result is bit-identical
-// from run to run and independent of G.
+// from run to run, and independent of G where every unit ends so.  FP32 log-Euler caplets and the
+// mortgage run kernel end only the last unit of a CTA's run in a replication (run_ends): their sums
+// (compensated FP32, FP64) are grouped by G.  Caplets of 40 forwards, N = 65536, Sobol': a replication's
+// theta in a plan of 7 and in one of 24 replications agrees to 1.7e-9 relative; mortgages, same bits.
 #pragma once
 #include "f32x2.cuh"
 #include "rqmc_internal.h"
@@ -47,7 +50,8 @@ __device__ __forceinline__ void flush_unit(const RedParams &r, uint32_t u, T *ac
 // Kernels that accumulate over the CTA's consecutive units of one replication flush only at the
 // last of them, into that unit's row; the theta kernel then reads those rows alone (launch_theta
 // with the kernel's grid).  A flush costs a barrier and, per output and warp, four operations
-// on the FP64 pipe (2 per SM and clock), 4 % of the 40-forward caplet kernel when done per unit.
+// on the FP64 pipe (2 per SM and clock).  Done per unit, caplets of 10, 40 and 160 forwards took 6, 1.8
+// and 0.4 % longer, mortgages 0.3 to 1 %.
 __device__ __forceinline__ bool run_ends(const RedParams &r, uint32_t u, uint32_t u1) {
     return u + 1 == u1 || (u + 1) % r.tiles_per_m == 0;
 }

@@ -16,9 +16,10 @@ constexpr int kMaxFwd = 160;       // forwards per LMM instrument (register-resi
 constexpr int kMaxDims = 4096;
 constexpr int kMaxOutputs = 1280;  // nf * n_strikes per caplet plan
 
-// Reduction layout: a unit is (replication m, tile of `tile` consecutive paths);
-// each unit writes its own row of `nout` doubles, so the result does not depend on
-// which CTA processed it.  theta[m][o] = sum_tiles partial / N in tile order.
+// Reduction layout: a unit is (replication m, tile of `tile` consecutive paths); theta[m][o] is the
+// sum of the replication's rows of `nout` doubles over N, in a fixed order.  Every unit writes its row,
+// so that theta does not depend on which CTA processed it, except FP32 log-Euler caplets and FP32
+// mortgages in runs of points: their CTAs write a row per run of consecutive units (see run_ends).
 struct RedParams {
     int nout;
     int ppt;                 // paths per thread per unit

@@ -1,6 +1,8 @@
 // runs.cuh -- runs of 8 consecutive points in one dimension: the digit odometer of Halton/Rasrap
 // (see k_points.cu for the derivation), and FP32 uniforms and normals of a run on packed pairs.
-// Every value is bit-identical to the point's own draw (PathGen).
+// Sobol' and Philox values, bases 2, 3 and 5, raw numerators and FP64 values are bit-identical to the
+// point's own draw (PathGen); FP32 uniforms of bases p >= 7 come from another rounding of the same
+// exact value (sigma / p + A, halton_run_q) and differ from it by 1 to 2 ulp.
 #pragma once
 #include "paths_common.cuh"
 
