@@ -759,7 +759,7 @@ static rqmc_status make_adjoint(const rqmc_lmm_params *p, const double *strikes_
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    set_reduction(*pl, nout, kAdjointThreads, adjoint_ppt((uint64_t)N, M, sms));
+    set_reduction(*pl, nout, kAdjointThreads, adjoint_ppt((uint64_t)N, M, pl->nf_bucket, sms));
     AdjModel *md = new AdjModel();
     std::memset(md, 0, sizeof(AdjModel));
     pl->adjm = md;

@@ -277,12 +277,25 @@ inline int caplet64_threads(int n_fwd, int scheme) {
 // CTA size of the adjoint kernel: 64 threads of two paths, so that five CTAs (640 paths) fit the shared
 // memory of an SM with the state columns of an 80-forward strip.
 constexpr int kAdjointThreads = 64;
-// Points per thread and unit of an adjoint plan: two (one pass) for the balance of plans of few units,
-// up to eight, which spares partial rows and flushes, while 24 units per resident CTA (six per SM) remain.
-inline int adjoint_ppt(uint64_t N, int M, int sms) {
-    int ppt = 8;
-    while (ppt > 2 && N * (uint64_t)M < 24ull * 6 * (uint64_t)sms * kAdjointThreads * (uint64_t)ppt) ppt /= 2;
-    return ppt;
+// Points per thread and unit of an adjoint plan: 2 (one pass), 4 or 8, the shape with the least time by a
+// count: the rounds of units that the resident CTAs (five or six per SM) take, each its passes and a
+// flush of about a twentieth of a pass.  More points per unit spare flushes and partial rows, fewer leave
+// less of the last round idle.  Measured, ms at 2 | 4 | 8: 80 forwards, two factors, N M = 2^21 13.70 |
+// 13.55 | 14.53, 2^23 54.8 | 54.7 | 54.2; 40, two factors, 2^20 1.86 | 1.99 | 2.17; 10 forwards, 2^22 1.00 |
+// 0.93 | 0.89, 2^20 0.255 | 0.257 | 0.288.
+inline int adjoint_ppt(uint64_t N, int M, int nf_bucket, int sms) {
+    const uint64_t cap = (nf_bucket == 40 ? 6ull : 5ull) * (uint64_t)sms;
+    uint64_t least = ~0ull;
+    int best = 2;
+    for (int ppt = 2; ppt <= 8; ppt *= 2) {
+        const uint64_t tile = (uint64_t)kAdjointThreads * (uint64_t)ppt, units = (N + tile - 1) / tile * (uint64_t)M;
+        const uint64_t cost = (units + cap - 1) / cap * (10ull * (uint64_t)ppt + 1);   // a pass of two points: 20
+        if (cost <= least) {
+            least = cost;
+            best = ppt;
+        }
+    }
+    return best;
 }
 
 // ---- the caller's initial curve as forwards (eq. BL for bond prices); p points into itself
