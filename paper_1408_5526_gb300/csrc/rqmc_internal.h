@@ -280,9 +280,9 @@ constexpr int kAdjointThreads = 64;
 // Points per thread and unit of an adjoint plan: 2 (one pass), 4 or 8, the shape with the least time by a
 // count: the rounds of units that the resident CTAs (five or six per SM) take, each its passes and a
 // flush of about a twentieth of a pass.  More points per unit spare flushes and partial rows, fewer leave
-// less of the last round idle.  Measured (with an earlier, slower flush), ms at 2 | 4 | 8: 80 forwards, two factors, N M = 2^21 13.70 |
-// 13.55 | 14.53, 2^23 54.8 | 54.7 | 54.2; 40, two factors, 2^20 1.86 | 1.99 | 2.17; 10 forwards, 2^22 1.00 |
-// 0.93 | 0.89, 2^20 0.255 | 0.257 | 0.288.
+// less of the last round idle.  Measured, Sobol', ms at 2 | 4 | 8: 80 forwards, two factors, N M = 2^21 13.59 | 13.49 | 14.38,
+// 2^23 54.0 | 54.2 | 53.6; 40, two factors, 2^20 1.76 | 1.92 | 2.15; 10 forwards, 2^22 0.92 | 0.86 | 0.82,
+// 2^20 0.253 | 0.257 | 0.285.
 inline int adjoint_ppt(uint64_t N, int M, int nf_bucket, int sms) {
     const uint64_t cap = (nf_bucket == 40 ? 6ull : 5ull) * (uint64_t)sms;
     uint64_t least = ~0ull;
